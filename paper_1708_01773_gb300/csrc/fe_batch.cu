@@ -67,7 +67,7 @@ constexpr int kWarps = kThreads / 32;
 // RHS entries are formed separately (rhs_rows).
 template <int NL>
 __device__ void row_slots(const ScatterParams& p, int64_t r, int lane, float2* acc) {
-  using S = SlotScatter<NL, 1, true>;
+  using S = SlotScatter<NL, 1, KeWritten::kSameLaunch>;
   const int64_t s0 = p.slot_ptr[r];
   const int ns = int(p.slot_ptr[r + 1] - s0);
   const int64_t k0 = p.row_ptr[r];

@@ -1446,12 +1446,19 @@ __device__ __forceinline__ void cell_block(const CellParams& prm, int64_t e0, in
   }
 }
 
-// Read-only loads of the scatter: through the non-coherent read-only path,
-// or, for data written earlier in the same launch by other blocks (the
-// batched driver), bypassing L1 (ld.global.cg).
-template <bool CG, typename T>
-__device__ __forceinline__ T ld_ro(const T* p) {
-  if constexpr (CG) return __ldcg(p); else return __ldg(p);
+// How a scatter reads the cell matrices, which depends on when they are written:
+// kBefore, by a kernel that ended before this launch began: the non-coherent
+// read-only path (ld.global.nc asks for data that nobody writes while the
+// reading grid exists); kOverlap, by a kernel that this launch overlaps and
+// waits for (griddepcontrol.wait): ordinary loads, which neither the compiler nor
+// the hardware may move before the wait; kSameLaunch, by other blocks of this
+// launch (the batched driver): bypassing L1 (ld.global.cg).
+enum class KeWritten { kBefore, kOverlap, kSameLaunch };
+template <KeWritten W, typename T>
+__device__ __forceinline__ T ld_ke(const T* p) {
+  if constexpr (W == KeWritten::kSameLaunch) return __ldcg(p);
+  else if constexpr (W == KeWritten::kOverlap) return *p;
+  else return __ldg(p);
 }
 
 // One batch of the slot-wise double-float scatter of k_scatter_slots (see
@@ -1460,8 +1467,9 @@ __device__ __forceinline__ T ld_ro(const T* p) {
 // a private dummy per lane at index `dummy`. The first contribution of a
 // nonzero (flag bit 15 of pos; every entry of slot 0) stores (v, 0); later
 // ones add with TwoSum.
-template <int NL, int R, bool CG = false>
+template <int NL, int R, KeWritten W = KeWritten::kBefore>
 struct SlotScatter {
+  static constexpr KeWritten kWritten = W;
   static constexpr int CH = (NL + 31) / 32;
   static constexpr int NBR = NL / R;  // local-row offset between the rows of one node
   static constexpr int LOADS = CH * (R + 1);
@@ -1483,10 +1491,10 @@ struct SlotScatter {
       const uint16_t* prow = pos + s * NL;
 #pragma unroll
       for (int c = 0; c < CH; ++c) {
-        const int k = int(ld_ro<CG>(prow + c * 32));
+        const int k = int(W == KeWritten::kSameLaunch ? __ldcg(prow + c * 32) : __ldg(prow + c * 32));
         kk[t][c] = (c < CH - 1 || c * 32 + lane < NL) ? k : dummy;
 #pragma unroll
-        for (int i = 0; i < R; ++i) x[t][c][i] = ld_ro<CG>(krow + i * NBR * p.nlp + c * 32);
+        for (int i = 0; i < R; ++i) x[t][c][i] = ld_ke<W>(krow + i * NBR * p.nlp + c * 32);
       }
     }
 #pragma unroll

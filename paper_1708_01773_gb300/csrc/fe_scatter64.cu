@@ -14,8 +14,9 @@ constexpr int kSlotGrab = 4;  // items per grab
 // accumulator is an FxChain, its sum and its exponent kept in two arrays of the
 // warp's shared memory: at least as accurate as FP64 additions, which this GPU
 // issues at 2 lanes per clock per SM.
-template <int NL, int R>
+template <int NL, int R, KeWritten W = KeWritten::kBefore>
 struct SlotScatter64 {
+  static constexpr KeWritten kWritten = W;
   static constexpr int CH = (NL + 31) / 32;
   static constexpr int NBR = NL / R;
   static constexpr int LOADS = CH * R;
@@ -38,7 +39,7 @@ struct SlotScatter64 {
         const bool in = c < CH - 1 || c * 32 + lane < NL;
         kk[t][c] = in ? int(__ldg(prow + c * 32)) : dummy;
 #pragma unroll
-        for (int i = 0; i < R; ++i) x[t][c][i] = in ? __ldg(krow + i * NBR * p.nlp + c * 32) : 0.0;
+        for (int i = 0; i < R; ++i) x[t][c][i] = in ? ld_ke<W>(krow + i * NBR * p.nlp + c * 32) : 0.0;
       }
     }
 #pragma unroll
@@ -232,12 +233,14 @@ constexpr int kSmallRowsPerSm = 320;
 //                   117,649 rows 74 / 93 -> 74 / 115
 // so the line is drawn at kSmallRowsPerSm rows per SM (48,640 on GB300).
 // Launched to overlap the cell kernel's end: only static data is read before
-// griddepcontrol.wait.
+// griddepcontrol.wait, and the cell kernel's data with ordinary loads.
 // Per nonzero the same terms in the same order as those kernels.
 template <int NL, typename TK>
 __global__ void __launch_bounds__(kScatterWarps * 32) k_scatter_small(ScatterParams p) {
   constexpr bool F64 = sizeof(TK) == 8;
-  using S = std::conditional_t<F64, SlotScatter64<NL, 1>, SlotScatter<NL, 1>>;
+  constexpr KeWritten W = KeWritten::kOverlap;
+  using S = std::conditional_t<F64, SlotScatter64<NL, 1, W>, SlotScatter<NL, 1, W>>;
+  static_assert(S::kWritten == KeWritten::kOverlap, "this grid overlaps the kernel that writes the cell matrices");
   extern __shared__ __align__(16) unsigned char sm[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t r = int64_t(blockIdx.x) * kScatterWarps + warp;
