@@ -439,7 +439,8 @@ int fe_compliance_work_size(const fe_dirichlet* d, int64_t* n_doubles);
  * Synchronises `stream` (the host checks convergence). Errors:
  * FE_ERR_NOT_CONVERGED (max_iter reached; u holds the last iterate),
  * FE_ERR_INVALID_ARG (also: the constrained matrix is not positive definite,
- * e.g. too few DOFs fixed), FE_ERR_CUDA. */
+ * e.g. too few DOFs fixed; the squared norms of the load or of the solve leave
+ * FP64's range), FE_ERR_CUDA. */
 int fe_compliance(fe_dirichlet* d, const double* coefficients, const double* body_force, fe_precision prec,
                   double rtol, int max_iter, double* work, double* u, double* compliance, double* dc_dcoef,
                   int* iterations, double* rel_residual, void* stream);

@@ -48,7 +48,7 @@ constexpr long long kPcgWait = 1ll << 31;  // clock cycles before a wait gives u
 // device scalars
 enum { S_RZ = 0, S_IT = 1, S_RR = 2, S_BB = 3, S_FLAG = 4, kScalars = 8 };
 // S_FLAG bits
-constexpr int kFlagNotSpd = 1, kFlagTimeout = 2;
+constexpr int kFlagNotSpd = 1, kFlagTimeout = 2, kFlagDiverged = 4;
 
 struct CgParams {
   int64_t n;
@@ -232,6 +232,9 @@ struct Exchange {
   }
 };
 
+// (on the integer bits, off the FP64 pipe)
+__device__ __forceinline__ bool is_finite(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+
 // a / b from 1 / b; at the ends of the exponent range, where 1 / b overflows or
 // loses bits (loads of the order of 1e-150), the division
 static __device__ __noinline__ double quotient_slow(double a, double b) { return a / b; }
@@ -241,8 +244,10 @@ __device__ __forceinline__ double quotient(double a, double b, double inv_b) {
 }
 
 // Up to n_it PCG iterations (see the head of this file), ending early at a
-// check (every kCheckEvery iterations) that finds ||r|| <= rtol ||b||, a sum
-// that is not finite or a matrix that is not positive definite. Cooperative
+// check (every kCheckEvery iterations) that finds ||r|| <= rtol ||b|| or a
+// matrix that is not positive definite, and at once where p.q, r.z or r.r is not
+// finite: such a sum does not recover, and no later residual may pass for a
+// converged one. Cooperative
 // launch: every block is resident. Virtual block vb owns rows
 // [n vb / nv, n (vb + 1) / nv).
 //
@@ -279,7 +284,7 @@ __global__ void __launch_bounds__(kPcgThreads, 1) k_pcg(CgParams p, int nv, int 
   // (thread 0's copies are the ones that count)
   double rz = p.s[S_RZ], rr = 0.0;
   const double bb = p.s[S_BB];
-  bool not_spd = false;
+  bool not_spd = false, diverged = false;
   auto row0 = [&](int vb) { return p.n * vb / nv; };
   // block sums of a and (TWO) b over the first `lim` threads (a multiple of 32)
   // in a fixed order, then the block's arrival
@@ -368,6 +373,7 @@ __global__ void __launch_bounds__(kPcgThreads, 1) k_pcg(CgParams p, int nv, int 
     const double inv_rz = warp == 0 ? reciprocal(rz) : 0.0;  // (thread 0's, while the others arrive)
     x.template finish<false>(got, bc, [&](double pq, double, double* o) {
       not_spd |= !(pq > 0.0) && rz > 0.0;
+      diverged |= !is_finite(pq);
       o[0] = pq > 0.0 ? quotient(rz, pq, reciprocal(pq)) : 0.0;
     });
     if (x.gave_up) break;
@@ -403,8 +409,9 @@ __global__ void __launch_bounds__(kPcgThreads, 1) k_pcg(CgParams p, int nv, int 
       o[0] = rz > 0.0 ? quotient(rz_new, rz, inv_rz) : 0.0;
       rz = rz_new;
       rr = rr_new;
+      diverged |= !is_finite(rz) || !is_finite(rr);
       const bool check = it % kCheckEvery == 0 || it == n_it;
-      o[1] = check && (not_spd || !(sqrt(fmax(0.0, rr) / bb) > rtol)) ? 1.0 : 0.0;
+      o[1] = diverged || (check && (not_spd || !(sqrt(rr / bb) > rtol))) ? 1.0 : 0.0;
     });
     if (x.gave_up || got[1] != 0.0) break;
     const double beta = got[0];
@@ -430,9 +437,9 @@ __global__ void __launch_bounds__(kPcgThreads, 1) k_pcg(CgParams p, int nv, int 
     p.s[S_RZ] = rz;
     p.s[S_RR] = rr;
     p.s[S_IT] = double(it);
-    if (not_spd || x.gave_up)
-      atomicOr(reinterpret_cast<unsigned long long*>(p.s + S_FLAG),
-               static_cast<unsigned long long>((not_spd ? kFlagNotSpd : 0) | (x.gave_up ? kFlagTimeout : 0)));
+    const int flags = (not_spd ? kFlagNotSpd : 0) | (diverged ? kFlagDiverged : 0) | (x.gave_up ? kFlagTimeout : 0);
+    if (flags)
+      atomicOr(reinterpret_cast<unsigned long long*>(p.s + S_FLAG), static_cast<unsigned long long>(flags));
   }
 }
 
@@ -504,6 +511,8 @@ int compliance_solve(const ComplianceArgs& a, cudaStream_t st) {
     uint64_t flag = 0;
     std::memcpy(&flag, &hs[S_FLAG], sizeof(flag));
     if (flag & kFlagNotSpd) return set_error(FE_ERR_INVALID_ARG, "compliance: a diagonal entry is not positive");
+    if (!std::isfinite(bb) || !std::isfinite(hs[S_RZ]))
+      return set_error(FE_ERR_INVALID_ARG, "compliance: the squared norms of the load are not finite");
     int it = 0;
     double rel = 0.0;
     if (bb > 0.0) {
@@ -540,8 +549,8 @@ int compliance_solve(const ComplianceArgs& a, cudaStream_t st) {
         if (flag & kFlagTimeout) return set_error(FE_ERR_TIMEOUT, "compliance: a bounded device wait gave up");
         if (flag & kFlagNotSpd) return set_error(FE_ERR_INVALID_ARG, "compliance: the constrained matrix is not positive definite");
         it += int(hs[S_IT]);
-        rel = std::sqrt(std::max(0.0, hs[S_RR]) / bb);
-        if (!std::isfinite(rel)) return set_error(FE_ERR_INVALID_ARG, "compliance: PCG diverged");
+        rel = std::sqrt(hs[S_RR] / bb);
+        if ((flag & kFlagDiverged) || !std::isfinite(rel)) return set_error(FE_ERR_INVALID_ARG, "compliance: PCG diverged");
       }
     }  // else b = 0: the initial x = 0 is the solution
     *a.iterations = it;
