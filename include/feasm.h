@@ -445,6 +445,14 @@ int fe_compliance(fe_dirichlet* d, const double* coefficients, const double* bod
                   double rtol, int max_iter, double* work, double* u, double* compliance, double* dc_dcoef,
                   int* iterations, double* rel_residual, void* stream);
 
+/* Self-test: fe_compliance in which a cooperative launch of more than
+ * max_blocks >= 1 blocks counts as refused, as it is in a process that may use
+ * only part of the GPU's multiprocessors. The iterations then run in fewer
+ * blocks, with the same sums whatever their number. */
+int fe_selftest_compliance(fe_dirichlet* d, const double* coefficients, const double* body_force, fe_precision prec,
+                           double rtol, int max_iter, double* work, double* u, double* compliance, double* dc_dcoef,
+                           int* iterations, double* rel_residual, int max_blocks, void* stream);
+
 /* Frees the constrained system (before its space). */
 void fe_dirichlet_destroy(fe_dirichlet* d);
 

@@ -371,9 +371,9 @@ int fe_compliance_work_size(const fe_dirichlet* d, int64_t* n_doubles) {
   return FE_OK;
 }
 
-int fe_compliance(fe_dirichlet* d, const double* coefficients, const double* body_force, fe_precision prec,
-                  double rtol, int max_iter, double* work, double* u, double* compliance, double* dc_dcoef,
-                  int* iterations, double* rel_residual, void* stream) {
+static int compliance_entry(fe_dirichlet* d, const double* coefficients, const double* body_force, fe_precision prec,
+                            double rtol, int max_iter, double* work, double* u, double* compliance, double* dc_dcoef,
+                            int* iterations, double* rel_residual, int max_blocks, void* stream) {
   if (!d || !body_force || !work || !compliance || (d->s->hs.n_dofs && !u) || (d->s->n_cells && !coefficients))
     return feasm::set_error(FE_ERR_INVALID_ARG, "NULL argument");
   if (d->s->host_only) return feasm::set_error(FE_ERR_INVALID_ARG, "host-only space cannot compute");
@@ -401,6 +401,7 @@ int fe_compliance(fe_dirichlet* d, const double* coefficients, const double* bod
   a.compliance = compliance;
   a.iterations = iterations ? iterations : &it_local;
   a.rel_residual = rel_residual ? rel_residual : &rel_local;
+  a.max_blocks = max_blocks;
   const int rc = feasm::compliance_solve(a, st);
   if (rc) return rc;
   if (dc_dcoef && s->n_cells) {
@@ -409,6 +410,21 @@ int fe_compliance(fe_dirichlet* d, const double* coefficients, const double* bod
     if (e != cudaSuccess) return cuda_fail(e, "compliance gradient");
   }
   return FE_OK;
+}
+
+int fe_compliance(fe_dirichlet* d, const double* coefficients, const double* body_force, fe_precision prec,
+                  double rtol, int max_iter, double* work, double* u, double* compliance, double* dc_dcoef,
+                  int* iterations, double* rel_residual, void* stream) {
+  return compliance_entry(d, coefficients, body_force, prec, rtol, max_iter, work, u, compliance, dc_dcoef, iterations,
+                          rel_residual, 0, stream);
+}
+
+int fe_selftest_compliance(fe_dirichlet* d, const double* coefficients, const double* body_force, fe_precision prec,
+                           double rtol, int max_iter, double* work, double* u, double* compliance, double* dc_dcoef,
+                           int* iterations, double* rel_residual, int max_blocks, void* stream) {
+  if (max_blocks < 1) return feasm::set_error(FE_ERR_INVALID_ARG, "max_blocks must be positive");
+  return compliance_entry(d, coefficients, body_force, prec, rtol, max_iter, work, u, compliance, dc_dcoef, iterations,
+                          rel_residual, max_blocks, stream);
 }
 
 void fe_dirichlet_destroy(fe_dirichlet* d) {

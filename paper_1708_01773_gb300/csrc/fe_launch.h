@@ -131,6 +131,7 @@ struct ComplianceArgs {
   double* compliance = nullptr;    // device scalar
   int* iterations = nullptr;       // host
   double* rel_residual = nullptr;  // host
+  int max_blocks = 0;              // > 0: cooperative launches of more blocks count as refused (self-test)
 };
 int64_t compliance_work_doubles(int64_t n_free, int64_t nnz);
 int compliance_solve(const ComplianceArgs& a, cudaStream_t st);

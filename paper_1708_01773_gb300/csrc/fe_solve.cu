@@ -534,14 +534,26 @@ int compliance_solve(const ComplianceArgs& a, cudaStream_t st) {
       const void* kern = res ? kernel(std::true_type()) : kernel(std::false_type());
       if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPcgThreads, 0);
       if (e != cudaSuccess || per_sm < 1) return set_error(FE_ERR_CUDA, "compliance: PCG launch");
-      const int grid = std::min(nv, nsm * per_sm);
+      int grid = std::min(nv, nsm * per_sm);
       rel = 1.0;
       while (it < a.max_iter && rel > a.rtol) {
         int n_it = std::min(kChunk, a.max_iter - it);
         double rtol = a.rtol;
         void* args[] = {&p, &nv, &n_it, &rtol};
+        auto launch = [&] {
+          if (a.max_blocks > 0 && grid > a.max_blocks) return cudaErrorCooperativeLaunchTooLarge;
+          return cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(kPcgThreads), args, 0, st);
+        };
         e = cudaMemsetAsync(p.part_b, 0xff, Exchange::kSets * kVirtual * 2 * sizeof(double), st);
-        if (e == cudaSuccess) e = cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(kPcgThreads), args, 0, st);
+        if (e == cudaSuccess) e = launch();
+        // a process that may use part of the SMs only: the form that keeps its vectors
+        // in memory, whose blocks loop over the virtual blocks, with as many as fit
+        while (e == cudaErrorCooperativeLaunchTooLarge && grid > 1) {
+          cudaGetLastError();
+          kern = kernel(std::false_type());
+          grid /= 2;
+          e = launch();
+        }
         if (e == cudaSuccess) e = cudaMemcpyAsync(hs.data(), p.s, kScalars * sizeof(double), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return set_error(FE_ERR_CUDA, "compliance: PCG iteration");

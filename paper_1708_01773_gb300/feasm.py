@@ -32,7 +32,7 @@ EXPORTS = [
     "fe_batch_assemble", "fe_batch_set_wait", "fe_batch_destroy", "fe_selftest_conversions", "fe_space_dof_points_host", "fe_mesh_locality_order", "fe_dirichlet_create", "fe_dirichlet_sizes",
     "fe_dirichlet_labels_host", "fe_dirichlet_csr_pattern_host", "fe_dirichlet_csr_pattern",
     "fe_dirichlet_permutation_host", "fe_dirichlet_lift_host", "fe_assemble_dirichlet", "fe_dirichlet_destroy",
-    "fe_compliance_work_size", "fe_compliance", "fe_space_block_offset", "fe_dg_create", "fe_dg_create_host",
+    "fe_compliance_work_size", "fe_compliance", "fe_selftest_compliance", "fe_space_block_offset", "fe_dg_create", "fe_dg_create_host",
     "fe_dg_sizes", "fe_dg_csr_pattern_host", "fe_dg_csr_pattern", "fe_dg_facets_host", "fe_dg_assemble",
     "fe_dg_destroy",
 ]
@@ -107,6 +107,7 @@ def lib() -> ctypes.CDLL:
         L.fe_dg_destroy.argtypes = [V]
         L.fe_dg_destroy.restype = None
         L.fe_compliance.argtypes = [V, V, V, I, D, I, V, V, V, V, P(I), P(D), V]
+        L.fe_selftest_compliance.argtypes = [V, V, V, I, D, I, V, V, V, V, P(I), P(D), I, V]
         L.fe_dirichlet_destroy.argtypes = [V]
         L.fe_dirichlet_destroy.restype = None
         for n in EXPORTS:
@@ -408,6 +409,16 @@ def fe_compliance(d: int, coefficients, body_force, prec: int, rtol: float, max_
     _check(lib().fe_compliance(d, _ptr(coefficients), f, prec, float(rtol), int(max_iter), _ptr(work),
                                _ptr(u), _ptr(compliance), _ptr(dc_dcoef), ctypes.byref(it), ctypes.byref(rel),
                                _stream(stream)), "fe_compliance")
+    return it.value, rel.value
+
+
+def fe_selftest_compliance(d: int, coefficients, body_force, prec: int, rtol: float, max_iter: int, work, u, compliance,
+                           max_blocks: int, stream=None):
+    """fe_compliance, without the gradient, in at most max_blocks blocks."""
+    it, rel = ctypes.c_int(), ctypes.c_double()
+    _check(lib().fe_selftest_compliance(d, _ptr(coefficients), _force(body_force), prec, float(rtol), int(max_iter),
+                                        _ptr(work), _ptr(u), _ptr(compliance), None, ctypes.byref(it),
+                                        ctypes.byref(rel), int(max_blocks), _stream(stream)), "fe_selftest_compliance")
     return it.value, rel.value
 
 

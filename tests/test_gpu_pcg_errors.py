@@ -57,3 +57,35 @@ def test_one_infinite_coefficient_is_an_error():
         with pytest.raises(feasm.FEError) as ei:
             dsys.compliance(torch.tensor(coef, device="cuda"), prec="fp64", rtol=1e-6)
         assert ei.value.code == -1
+
+
+@pytest.mark.parametrize("shape, order, problem", [((1, 1, 1), 1, 0), ((16, 17, 15), 1, 1), ((38, 38, 38), 1, 1),
+                                                   ((10, 9, 9), 2, 1)])
+def test_fewer_blocks_than_the_gpu_has(shape, order, problem):
+    """Cooperative launches above max_blocks are answered with the runtime's error
+    for a grid that does not fit. The residual is within the bound of the full
+    grid's (1.1 rtol), and the number of blocks does not change the result:
+    the partial sums belong to virtual blocks."""
+    prob, dsys = clamped(shape, order, problem)
+    coef = torch.tensor(prob.coef, device="cuda")
+    vals, f = dsys.assemble(coef, None, prec="fp64")
+    rp, col = dsys.pattern()
+    label = torch.tensor(dsys.labels().astype(np.int64), device="cuda")
+    rows = torch.repeat_interleave(torch.arange(dsys.n_free, device="cuda"), rp.diff())
+    work = torch.empty(feasm.fe_compliance_work_size(dsys.handle), dtype=torch.float64, device="cuda")
+    _, _, _, it_full, _ = dsys.compliance(coef, prec="fp64", rtol=1e-6)
+    results = []
+    for blocks in (1, 7, 75):
+        u = torch.full((dsys.space.n_dofs,), np.nan, dtype=torch.float64, device="cuda")
+        c = torch.empty(1, dtype=torch.float64, device="cuda")
+        it, rel = feasm.fe_selftest_compliance(dsys.handle, coef, prob.force, feasm.PRECISIONS["fp64"], 1e-6, 20000,
+                                               work, u, c, blocks)
+        x = torch.zeros(dsys.n_free, dtype=torch.float64, device="cuda")
+        x[label[label >= 0]] = u[label >= 0]
+        r = f.clone().index_add_(0, rows, -vals * x[col.long()])
+        assert rel <= 1e-6 and float(r.norm()) <= 1.1e-6 * float(f.norm())
+        assert abs(it - it_full) <= 8  # one interval between checks: the sums' order differs
+        results.append((it, rel, u, c))
+    if dsys.n_free > 32:  # (fewer rows make one virtual block: the full grid, vectors in registers)
+        for it, rel, u, c in results[1:]:
+            assert (it, rel) == results[0][:2] and torch.equal(u, results[0][2]) and torch.equal(c, results[0][3])
