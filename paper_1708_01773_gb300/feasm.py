@@ -143,8 +143,9 @@ _Force = ctypes.c_double * 3
 
 
 def _force(body_force):
-    """The force as three doubles, repeated or cut to length (np.resize)."""
-    if type(body_force) is np.ndarray and body_force.ndim == 1 and body_force.size:
+    """The force as three doubles, repeated or cut to length (np.resize). Arrays of real
+    numbers in one dimension take a shorter way (small assemblies are bound by the host)."""
+    if type(body_force) is np.ndarray and body_force.ndim == 1 and body_force.size and body_force.dtype.kind in "fiub":
         v = body_force.tolist()
         n = len(v)
         return _Force(v[0], v[1 % n], v[2 % n])
