@@ -71,6 +71,62 @@ __device__ __forceinline__ void adjoint_partial(const AdjParams& p, int64_t e, d
   if (threadIdx.x == 0) p.partials[blockIdx.x] = red[0];
 }
 
+// Energy of one cell in the FP64 form (a: trilinear coefficients of the geometry, ue: u at the cell's DOFs).
+template <int P, int NC>
+__device__ __forceinline__ double cell_energy_fp64(const AdjParams& p, const double (&a)[21],
+                                                   const double (&ue)[NC * (P + 1) * (P + 1) * (P + 1)]) {
+  constexpr int NB = (P + 1) * (P + 1) * (P + 1);
+  double energy = 0.0;
+  for (int q = 0; q < p.nq; ++q) {
+    double cof[9], det;
+    geometry_at(a, p.xq[3 * q], p.xq[3 * q + 1], p.xq[3 * q + 2], cof, &det);
+    if (!(det > 0.0)) atomicOr(p.err, kErrNegJacobian);
+    // reference gradient of each component of u
+    double gr[NC][3];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) gr[c][0] = gr[c][1] = gr[c][2] = 0.0;
+    const double* dq = p.dphi + size_t(q) * NB * 3;
+#pragma unroll 4
+    for (int b = 0; b < NB; ++b) {
+      const double d0 = dq[3 * b], d1 = dq[3 * b + 1], d2 = dq[3 * b + 2];
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        const double uc = ue[c * NB + b];
+        gr[c][0] += uc * d0;
+        gr[c][1] += uc * d1;
+        gr[c][2] += uc * d2;
+      }
+    }
+    // physical gradient: (grad u)_{c,k} = sum_d gr[c][d] cof[k][d] / det
+    const double inv = 1.0 / det;
+    double cs[9];
+#pragma unroll
+    for (int t = 0; t < 9; ++t) cs[t] = cof[t] * inv;
+    double gu[NC][3];
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) gu[c][k] = gr[c][0] * cs[3 * k] + gr[c][1] * cs[3 * k + 1] + gr[c][2] * cs[3 * k + 2];
+    double dens;
+    if (NC == 1) {
+      dens = gu[0][0] * gu[0][0] + gu[0][1] * gu[0][1] + gu[0][2] * gu[0][2];
+    } else {
+      const double div = gu[0][0] + gu[1 % NC][1] + gu[2 % NC][2];
+      double ee = 0.0;
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int l = 0; l < 3; ++l) {
+          const double eps = 0.5 * (gu[k % NC][l] + gu[l % NC][k]);
+          ee += eps * eps;
+        }
+      dens = p.lam_hat * (div * div) + 2.0 * p.mu_hat * ee;
+    }
+    energy += p.w[q] * det * dens;
+  }
+  return energy;
+}
+
 template <int P, int NC, typename T>
 __global__ void __launch_bounds__(kAdjThreads) k_adjoint(AdjParams p) {
   constexpr int NB = (P + 1) * (P + 1) * (P + 1);
@@ -123,53 +179,7 @@ __global__ void __launch_bounds__(kAdjThreads) k_adjoint(AdjParams p) {
     T ue[NL];
 #pragma unroll
     for (int l = 0; l < NL; ++l) ue[l] = T(p.u[p.cell_dofs[e * NL + l]]);
-    for (int q = 0; q < p.nq; ++q) {
-      double cof[9], det;
-      geometry_at(a, p.xq[3 * q], p.xq[3 * q + 1], p.xq[3 * q + 2], cof, &det);
-      if (!(det > 0.0)) atomicOr(p.err, kErrNegJacobian);
-      // reference gradient of each component of u
-      T gr[NC][3];
-#pragma unroll
-      for (int c = 0; c < NC; ++c) gr[c][0] = gr[c][1] = gr[c][2] = T(0);
-      const double* dq = p.dphi + size_t(q) * NB * 3;
-#pragma unroll 4
-      for (int b = 0; b < NB; ++b) {
-        const T d0 = T(dq[3 * b]), d1 = T(dq[3 * b + 1]), d2 = T(dq[3 * b + 2]);
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          const T uc = ue[c * NB + b];
-          gr[c][0] += uc * d0;
-          gr[c][1] += uc * d1;
-          gr[c][2] += uc * d2;
-        }
-      }
-      // physical gradient: (grad u)_{c,k} = sum_d gr[c][d] cof[k][d] / det
-      const double inv = 1.0 / det;
-      T cs[9];
-#pragma unroll
-      for (int t = 0; t < 9; ++t) cs[t] = T(cof[t] * inv);
-      T gu[NC][3];
-#pragma unroll
-      for (int c = 0; c < NC; ++c)
-#pragma unroll
-        for (int k = 0; k < 3; ++k) gu[c][k] = gr[c][0] * cs[3 * k] + gr[c][1] * cs[3 * k + 1] + gr[c][2] * cs[3 * k + 2];
-      double dens;
-      if (NC == 1) {
-        dens = double(gu[0][0] * gu[0][0] + gu[0][1] * gu[0][1] + gu[0][2] * gu[0][2]);
-      } else {
-        const T div = gu[0][0] + gu[1 % NC][1] + gu[2 % NC][2];
-        T ee = T(0);
-#pragma unroll
-        for (int k = 0; k < 3; ++k)
-#pragma unroll
-          for (int l = 0; l < 3; ++l) {
-            const T eps = T(0.5) * (gu[k % NC][l] + gu[l % NC][k]);
-            ee += eps * eps;
-          }
-        dens = p.lam_hat * double(div * div) + 2.0 * p.mu_hat * double(ee);
-      }
-      energy += p.w[q] * det * dens;
-    }
+    energy = cell_energy_fp64<P, NC>(p, a, ue);
     p.g[e] = p.grad_scale * energy;
     }
   }
@@ -190,13 +200,40 @@ __global__ void k_sum_partials(const double* partials, int n, double* out) {
   if (threadIdx.x == 0) *out = red[0];
 }
 
+// 2^-k with |x| 2^-k in [1, 2) for the largest |x| of n values (1 where that is
+// zero or not finite), k added to `sum` `times` times; exact.
+__device__ __forceinline__ void scale_to_one(double* x, int n, int times, int* sum) {
+  double m = 0.0;
+  for (int i = 0; i < n; ++i) m = fmax(m, fabs(x[i]));
+  const int k = m > 0.0 && m < INFINITY ? ilogb(m) : 0;
+  for (int i = 0; i < n; ++i) x[i] = scalbn(x[i], -k);
+  *sum += times * k;
+}
+
+// The same, out of line, for the cells that k_adjoint_q1 does not take: u and the
+// geometry scaled by powers of two, so that only the result may leave the range.
+template <int NC>
+static __device__ __noinline__ double cell_energy_scaled(const AdjParams& p, int64_t e) {
+  double a[21], ue[NC * 8];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) trilinear_coefficients(p.xv + e * 24, k, a);
+  for (int l = 0; l < NC * 8; ++l) ue[l] = p.u[p.cell_dofs[e * NC * 8 + l]];
+  int k = 0;
+  scale_to_one(a, 21, 1, &k);
+  scale_to_one(ue, NC * 8, 2, &k);
+  return scalbn(cell_energy_fp64<1, NC>(p, a, ue), k);
+}
+
 // Q1 with the 2^3 rule. The displacement's reference gradient has the same
 // trilinear form as the Jacobian, so both take their columns from the monomial
 // coefficients, each column once per pair of 1D points (column d depends on two
 // of the coordinates): 22 multiply-adds per component and cell instead of 72
 // (or 72 more for the gradient from the nodes). FP64 form: the physical
 // gradient times det J from the cofactors, so that 1 / det J enters once per
-// point, as an FP32 estimate with one cubic correction (3 FP64 operations).
+// point, as an FP32 estimate with one cubic correction (3 FP64 operations). That
+// squares u h^2 instead of u / h: a cell where the former leaves 2^+-440 or det J
+// 2^+-900 (found on the exponents, off the FP64 pipe) takes the general form with
+// u and the geometry scaled.
 // FP32 form: the strain as in k_adjoint, bit for bit but for the rounding of
 // the Jacobian. Bound by the FP64 pipe (2 lanes per clock per SM): about 760
 // FP64 operations per cell and 300 in the FP32 form, after 1,400 and 400.
@@ -221,6 +258,16 @@ struct Q1Columns {
       c2[1][y] = fma(t1, g1, t0);
     }
   }
+  // 0 if the component is the same at every node
+  __device__ __forceinline__ uint32_t bits() const {
+    uint32_t m = 0;
+    auto put = [&](double x) { m |= (uint32_t(__double2hiint(x)) & 0x7fffffffu) | uint32_t(__double2loint(x)); };
+#pragma unroll
+    for (int i = 0; i < 6; ++i) put(a[i]);
+    put(c2[0][0]);
+    put(c2[1][1]);
+    return m;
+  }
   // columns 0 at (y, z) and 1 at (x, z) for the given z
   __device__ __forceinline__ void slab(double z, double g0, double g1, double (&c0)[2], double (&c1)[2]) const {
     const double t1 = fma(a[5], z, a[2]), t0 = fma(a[3], z, a[0]), s0 = fma(a[4], z, a[1]);
@@ -232,7 +279,7 @@ struct Q1Columns {
 };
 
 template <int NC, typename T>
-__global__ void __launch_bounds__(kAdjThreads) k_adjoint_q1(AdjParams p) {
+__global__ void __launch_bounds__(kAdjThreads) k_adjoint_q1(const __grid_constant__ AdjParams p) {
   constexpr bool F32 = std::is_same<T, float>::value;
   constexpr int NL = NC * 8;
   __shared__ double red[kAdjThreads];
@@ -260,6 +307,16 @@ __global__ void __launch_bounds__(kAdjThreads) k_adjoint_q1(AdjParams p) {
       }
     }
     const float lh = d2f_rn(p.lam_hat), mh2 = 2.f * d2f_rn(p.mu_hat);
+    // high words: below lo a nonzero gradient, above hi any one is out of range
+    uint32_t lo = 0;
+    if constexpr (!F32) {
+      uint32_t nz = 0;
+#pragma unroll
+      for (int c = 0; c < NC; ++c) nz |= U[F32 ? 0 : c].bits();
+      lo = nz != 0 ? uint32_t(1023 - 440) << 20 : 0u;
+    }
+    constexpr uint32_t hi = uint32_t(1023 + 440) << 20;
+    bool odd = false;
 #pragma unroll 1
     for (int iz = 0; iz < 2; ++iz) {
       const double z = iz ? g1 : g0;
@@ -318,6 +375,13 @@ __global__ void __launch_bounds__(kAdjThreads) k_adjoint_q1(AdjParams p) {
 #pragma unroll
               for (int k = 0; k < 3; ++k)
                 gu[c][k] = U0[c][iy] * cof[3 * k] + U1[c][ix] * cof[3 * k + 1] + U[F32 ? 0 : c].c2[ix][iy] * cof[3 * k + 2];
+            uint32_t top = 0;
+#pragma unroll
+            for (int c = 0; c < NC; ++c)
+#pragma unroll
+              for (int k = 0; k < 3; ++k) top = max(top, uint32_t(__double2hiint(gu[c][k])) & 0x7fffffffu);
+            const uint32_t dh = uint32_t(__double2hiint(det)) & 0x7fffffffu;
+            odd |= top < lo || top > hi || dh - (uint32_t(1023 - 900) << 20) > (uint32_t(1800) << 20);
             double dens;
             if constexpr (NC == 1) {
               dens = gu[0][0] * gu[0][0] + gu[0][1] * gu[0][1] + gu[0][2] * gu[0][2];
@@ -331,6 +395,9 @@ __global__ void __launch_bounds__(kAdjThreads) k_adjoint_q1(AdjParams p) {
             energy = fma(p.w[q] * reciprocal(det), dens, energy);
           }
         }
+    }
+    if constexpr (!F32) {
+      if (odd) energy = cell_energy_scaled<NC>(p, e);
     }
     p.g[e] = p.grad_scale * energy;
   }
