@@ -633,9 +633,8 @@ struct FixedFacetLayout {
     int2 w[2][NQF][3];   // dS (cof^T n / det) along the face's normal axis and its two other axes
     int2 ds[NQF];        // dS
     int perm[2][NQF];    // the point's index in the side's own face rule
-    int ew, ey;          // scales: |w| < 2^ew, dS < 2^ey
+    int ew[2][2], ey;    // scales: |w| < 2^ew per side and kind of axis (normal, the two others), dS < 2^ey
     int odd;             // out of range: the products are NaN
-    int pad;
   };
   static constexpr size_t PT = 0;
   static constexpr size_t TAB = PT + 2 * ((sizeof(Points) + 15) & ~size_t(15));      // int2 [4][NQF][NBF]
@@ -658,8 +657,8 @@ __device__ __forceinline__ uint8_t face_node(int f, int a) {
 }
 
 // Point data of facet id for the fixed-point products (all 32 lanes of the
-// point warp): the geometry of facet_points, the weights dS cof^T n / det and
-// dS as integers under one scale each, and each point's index in the sides' own
+// point warp): the geometry of facet_points, the weights dS cof^T n / det as
+// integers under one scale per side and kind of axis, dS under one, and each point's index in the sides' own
 // face rules.
 template <int P>
 __device__ __forceinline__ void facet_points_fixed(const FacetParams& fp, int64_t id, typename FixedFacetLayout<P>::Points* b,
@@ -720,22 +719,39 @@ __device__ __forceinline__ void facet_points_fixed(const FacetParams& fp, int64_
   const double wn = d == 0 ? w[0] : d == 1 ? w[1] : w[2];
   const double ws = d == 0 ? w[1] : w[0], wt = d == 2 ? w[1] : w[2];
   auto top = [](double x) { return __double2hiint(x) & 0x7fffffff; };
-  const int mw = __reduce_max_sync(kFull, act ? max(top(wn), max(top(ws), top(wt))) : 0) >> 20;
+  // one scale per side and kind of axis: the weights go with 1 / (the cell's
+  // extent along the axis), which may differ by any factor between the two
+  // cells, and the rows of a cell's nodes off the face hold nothing of the other
+  int ew[2][2];
+  bool odd = false;
+#pragma unroll
+  for (int sd = 0; sd < 2; ++sd) {
+    const bool mine = act && side == sd;
+    const int mn = __reduce_max_sync(kFull, mine ? top(wn) : 0) >> 20;
+    const int mt = __reduce_max_sync(kFull, mine ? max(top(ws), top(wt)) : 0) >> 20;
+    ew[sd][0] = mn - 1022;
+    // (the tangential terms add to the normal ones: below 2^-400 of those they are nothing)
+    ew[sd][1] = max(mt - 1022, max(mn - 1422, 150 - 1022));
+    odd |= sd < f.ns && (mn < 150 || mn > 1900 || mt > 1900);
+  }
   const int my = __reduce_max_sync(kFull, act ? top(dsq) : 0) >> 20;
-  const int ew = mw - 1022, ey = my - 1022;
+  const int ey = my - 1022;
+  odd |= my < 150 || my > 1900;
   if (act) {
-    b->w[side][q][0] = fix_limbs<30>(fix_quantise(wn, 60 - ew));
-    b->w[side][q][1] = fix_limbs<30>(fix_quantise(ws, 60 - ew));
-    b->w[side][q][2] = fix_limbs<30>(fix_quantise(wt, 60 - ew));
+    const int en = side ? ew[1][0] : ew[0][0], et = side ? ew[1][1] : ew[0][1];
+    b->w[side][q][0] = fix_limbs<30>(fix_quantise(wn, 60 - en));
+    b->w[side][q][1] = fix_limbs<30>(fix_quantise(ws, 60 - et));
+    b->w[side][q][2] = fix_limbs<30>(fix_quantise(wt, 60 - et));
     if (side == 0) b->ds[q] = fix_limbs<30>(fix_quantise(dsq, 60 - ey));
     b->perm[side][q] = d == 0 ? at[1] + N1 * at[2] : d == 1 ? at[0] + N1 * at[2] : at[0] + N1 * at[1];
   }
   const double pen = fp.gamma * reciprocal(ar);
   if (lane == 0) {
     b->pen = pen;
-    b->ew = ew;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) b->ew[k >> 1][k & 1] = ew[k >> 1][k & 1];
     b->ey = ey;
-    b->odd = mw < 150 || mw > 1900 || my < 150 || my > 1900;
+    b->odd = odd;
   }
 }
 
@@ -836,8 +852,8 @@ __global__ void __launch_bounds__(128) k_dg_facets_fixed(FacetParams fp) {
         // X scaled by -s_a / 2 (boundary: -1), Y by s_a s_b
         const int h = f.interior ? 1 : 0;
         const int64_t ia = a.get(ga), ib = b.get(gb), iy = y.get(gy);
-        double A = fix_to_double(sa ? ia : -ia, fix_exponent(pt->ew + 2 * fp.fix_lp - 56 - ga - h));
-        double Bt = fix_to_double(sa ? ib : -ib, fix_exponent(pt->ew + fp.fix_lp + fp.fix_ld - 56 - gb - h));
+        double A = fix_to_double(sa ? ia : -ia, fix_exponent(pt->ew[sb][0] + 2 * fp.fix_lp - 56 - ga - h));
+        double Bt = fix_to_double(sa ? ib : -ib, fix_exponent(pt->ew[sb][1] + fp.fix_lp + fp.fix_ld - 56 - gb - h));
         double Yv = fix_to_double(sa == sb ? iy : -iy, fix_exponent(pt->ey + 2 * fp.fix_lp - 56 - gy));
         if (odd) A = Bt = Yv = __longlong_as_double(0x7ff8000000000000ll);
         const int fs = sb ? f.face[1] % 2 : f.face[0] % 2;  // the face layer of side sb
