@@ -627,6 +627,7 @@ __global__ void __launch_bounds__(128) k_dg_facets(FacetParams fp) {
 template <int P>
 struct FixedFacetLayout {
   static constexpr int N1 = P + 1, NB = N1 * N1 * N1, NQF = N1 * N1, NBF = N1 * N1;
+  // (odd_facets puts doubles in the place of w and ds)
   struct Points {
     FacetOut out;
     double pen;          // gamma / |F|
@@ -634,7 +635,7 @@ struct FixedFacetLayout {
     int2 ds[NQF];        // dS
     int perm[2][NQF];    // the point's index in the side's own face rule
     int ew[2][2], ey;    // scales: |w| < 2^ew per side and kind of axis (normal, the two others), dS < 2^ey
-    int odd;             // out of range: the products are NaN
+    int odd;             // out of range: left to odd_facets
   };
   static constexpr size_t PT = 0;
   static constexpr size_t TAB = PT + 2 * ((sizeof(Points) + 15) & ~size_t(15));      // int2 [4][NQF][NBF]
@@ -656,26 +657,11 @@ __device__ __forceinline__ uint8_t face_node(int f, int a) {
   return uint8_t(c | (m << 4));
 }
 
-// Point data of facet id for the fixed-point products (all 32 lanes of the
-// point warp): the geometry of facet_points, the weights dS cof^T n / det as
-// integers under one scale per side and kind of axis, dS under one, and each point's index in the sides' own
-// face rules.
+// Reference point (qs, qt) of the face rule on the given side, and the index of each coordinate among the 1D points.
 template <int P>
-__device__ __forceinline__ void facet_points_fixed(const FacetParams& fp, int64_t id, typename FixedFacetLayout<P>::Points* b,
-                                                   double* aco, int lane) {
-  using L = FixedFacetLayout<P>;
-  constexpr int N1 = L::N1, NB = L::NB, NQF = L::NQF;
-  static_assert(2 * NQF <= 32, "one lane per (side, point)");
-  const FacetRef f = facet_ref(fp, id);
-  if (lane < 3 * f.ns) trilinear_coefficients(fp.xv + f.cell[lane / 3] * 24, lane % 3, aco + (lane / 3) * 21);
-  if (f.interior && lane >= 30)
-    facet_out<NB>(fp, lane == 31 ? f.cell[1] : f.cell[0], lane == 31 ? f.face[1] : f.face[0], lane - 30, &b->out);
-  __syncwarp();
-  const bool act = lane < f.ns * NQF;
-  const int side = act ? lane / NQF : 0, q = lane % NQF, qs = q % N1, qt = q / N1;
+__device__ __forceinline__ void face_point(const FacetParams& fp, const FacetRef& f, int side, int qs, int qt, double (&xh)[3],
+                                           int (&at)[3]) {
   const double s = fp.gx[qs], tt = fp.gx[qt];
-  double xh[3];
-  int at[3];  // index of each coordinate among the 1D points
   const int d = side ? f.face[1] / 2 : f.face[0] / 2;
   const double fv = double(side ? f.face[1] % 2 : f.face[0] % 2);
   if (side == 0) {
@@ -696,6 +682,64 @@ __device__ __forceinline__ void facet_points_fixed(const FacetParams& fp, int64_
       at[k] = d1 > 0 ? qs : d1 < 0 ? P - qs : d2 > 0 ? qt : P - qt;
     }
   }
+}
+
+__device__ __forceinline__ double raw_double(int2 x) { return __hiloint2double(x.y, x.x); }
+__device__ __forceinline__ int2 raw_int2(double x) { return make_int2(__double2loint(x), __double2hiint(x)); }
+
+// The weights of a facet out of the fixed-point range (all 32 lanes of a product
+// warp), as plain doubles: the normal scaled by a power of two before it is
+// squared, and of unit length before the products.
+template <int P>
+__device__ __forceinline__ void facet_weights_fp64(const FacetParams& fp, const FacetRef& f,
+                                                   typename FixedFacetLayout<P>::Points* b, int lane) {
+  constexpr int N1 = P + 1, NQF = N1 * N1;
+  const bool act = lane < f.ns * NQF;
+  const int side = act ? lane / NQF : 0, q = lane % NQF, qs = q % N1, qt = q / N1, d = f.face[side] / 2, dp = f.face[0] / 2;
+  const double gww = fp.gw[qs] * fp.gw[qt];
+  double a[21], xh[3], cof[9], det, n[3], w[3];
+  int at[3];
+  for (int k = 0; k < 3; ++k) trilinear_coefficients(fp.xv + f.cell[side] * 24, k, a);
+  face_point<P>(fp, f, side, qs, qt, xh, at);
+  facet_geometry(a, xh[0], xh[1], xh[2], cof, &det);
+  for (int k = 0; k < 3; ++k) n[k] = __shfl_sync(kFull, flip(cof[3 * k + dp], f.face[0] % 2 == 0), q);
+  const double big = fmax(fabs(n[0]), fmax(fabs(n[1]), fabs(n[2])));
+  const int e = big > 0.0 && big < INFINITY ? ilogb(big) : 0;
+  for (int k = 0; k < 3; ++k) n[k] = scalbn(n[k], -e);
+  const double len = sqrt(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]), rdet = 1.0 / det, ds = scalbn(len, e) * gww;
+  for (int k = 0; k < 3; ++k)
+    w[k] = (cof[k] * (n[0] / len) + cof[3 + k] * (n[1] / len) + cof[6 + k] * (n[2] / len)) * rdet * ds;
+  if (act) {
+    b->w[side][q][0] = raw_int2(w[d]);
+    b->w[side][q][1] = raw_int2(w[d == 0 ? 1 : 0]);
+    b->w[side][q][2] = raw_int2(w[d == 2 ? 1 : 2]);
+    if (side == 0) b->ds[q] = raw_int2(ds);
+  }
+  const double ar = low_lanes_sum<NQF>(lane < NQF ? ds : 0.0);
+  if (lane == 0) b->pen = fp.gamma / ar;
+}
+
+// Point data of facet id for the fixed-point products (all 32 lanes of the
+// point warp): the geometry of facet_points, the weights dS cof^T n / det as
+// integers under one scale per side and kind of axis, dS under one, and each point's index in the sides' own
+// face rules.
+template <int P>
+__device__ __forceinline__ void facet_points_fixed(const FacetParams& fp, int64_t id, typename FixedFacetLayout<P>::Points* b,
+                                                   double* aco, int lane) {
+  using L = FixedFacetLayout<P>;
+  constexpr int N1 = L::N1, NB = L::NB, NQF = L::NQF;
+  static_assert(2 * NQF <= 32, "one lane per (side, point)");
+  const FacetRef f = facet_ref(fp, id);
+  if (lane < 3 * f.ns) trilinear_coefficients(fp.xv + f.cell[lane / 3] * 24, lane % 3, aco + (lane / 3) * 21);
+  if (f.interior && lane >= 30)
+    facet_out<NB>(fp, lane == 31 ? f.cell[1] : f.cell[0], lane == 31 ? f.face[1] : f.face[0], lane - 30, &b->out);
+  __syncwarp();
+  const bool act = lane < f.ns * NQF;
+  const int side = act ? lane / NQF : 0, q = lane % NQF, qs = q % N1, qt = q / N1;
+  const int d = side ? f.face[1] / 2 : f.face[0] / 2;
+  double xh[3];
+  int at[3];
+  face_point<P>(fp, f, side, qs, qt, xh, at);
   double cof[9], det;
   facet_geometry(aco + side * 21, xh[0], xh[1], xh[2], cof, &det);
   if (act && !(det > 0.0)) atomicOr(fp.err, kErrNegJacobian);
@@ -755,6 +799,80 @@ __device__ __forceinline__ void facet_points_fixed(const FacetParams& fp, int64_
   }
 }
 
+// The block's facets that are out of the fixed-point range, in plain FP64 with the
+// same steps as k_dg_facets_fixed, one facet at a time by all threads of the block.
+template <int P>
+static __device__ __noinline__ void odd_facets(const FacetParams& fp, unsigned char* sm, double* aco) {
+  using L = FixedFacetLayout<P>;
+  constexpr int N1 = L::N1, NB = L::NB, NQF = L::NQF, NBF = L::NBF;
+  auto* pt = reinterpret_cast<typename L::Points*>(sm + L::PT);
+  const int2* tab = reinterpret_cast<const int2*>(sm + L::TAB);
+  double* R = reinterpret_cast<double*>(sm + L::R);
+  double* X = reinterpret_cast<double*>(sm + L::X);
+  double* Y = reinterpret_cast<double*>(sm + L::Y);
+  double* XB = reinterpret_cast<double*>(sm + L::XB);
+  const double* Dn = reinterpret_cast<const double*>(sm + L::DN);
+  const uint8_t* nodes = sm + L::NODES;
+  const int t = threadIdx.x, nt = blockDim.x, lp = fp.fix_lp, ld = fp.fix_ld;
+  auto value = [](int2 l, int scale) { return scalbn(double((int64_t(l.x) << 30) + l.y), -scale); };
+  for (int64_t id = blockIdx.x; id < fp.n_int + fp.n_bnd; id += gridDim.x) {
+    if (t < 32) facet_points_fixed<P>(fp, id, pt, aco, t);
+    __syncthreads();
+    if (pt->odd) {
+      const FacetRef f = facet_ref(fp, id);
+      const int ns = f.ns, side_bit[2] = {f.face[0] % 2, f.face[1] % 2};
+      if (t < 32) facet_weights_fp64<P>(fp, f, pt, t);
+      __syncthreads();
+      for (int i = t; i < ns * NQF * NBF; i += nt) {
+        const int c = i % NBF, sq = i / NBF, side = sq / NQF, q = sq % NQF;
+        const int2* row = tab + NQF * NBF + pt->perm[side][q] * NBF + c;
+        const double ph = value(row[0], 60 - lp), ps = value(row[NQF * NBF], 60 - ld), pq = value(row[2 * NQF * NBF], 60 - ld);
+        R[i * 3] = raw_double(pt->w[side][q][0]) * ph;
+        R[i * 3 + 1] = raw_double(pt->w[side][q][1]) * ps + raw_double(pt->w[side][q][2]) * pq;
+        R[i * 3 + 2] = raw_double(pt->ds[q]) * ph;
+      }
+      __syncthreads();
+      for (int i = t; i < ns * ns * NBF * NBF; i += nt) {
+        const int c2 = i % NBF, rest = i / NBF, c = rest % NBF, blk = rest / NBF, sa = blk >> 1, sb = blk & 1;
+        double s[3] = {0.0, 0.0, 0.0};
+        for (int q = 0; q < NQF; ++q) {
+          const double ph = value(tab[pt->perm[sa][q] * NBF + c], 59 - lp);
+          const double* r = R + ((sb * NQF + q) * NBF + c2) * 3;
+          for (int k = 0; k < 3; ++k) s[k] = fma(ph, r[k], s[k]);
+        }
+        const double half = (sa ? 1.0 : -1.0) * (f.interior ? 0.5 : 1.0);
+        const int fs = side_bit[sb];
+        double* x = X + (blk * NBF + c) * NB + c2;
+        for (int m = 0; m < N1; ++m) x[m * NBF] = Dn[fs * N1 + m] * (half * s[0]);
+        x[fs * P * NBF] += half * s[1];
+        Y[i] = sa == sb ? s[2] : -s[2];
+      }
+      __syncthreads();
+      for (int i = t; i < ns * ns * NBF * NBF; i += nt) {
+        const int c2 = i % NBF, rest = i / NBF, c = rest % NBF, blk = rest / NBF, sa = blk >> 1, sb = blk & 1;
+        XB[i] = pt->pen * Y[i] + (fp.tau * X[(((sb << 1) | sa) * NBF + c2) * NB + side_bit[sa] * P * NBF + c] +
+                                  X[(blk * NBF + c) * NB + side_bit[sb] * P * NBF + c2]);
+      }
+      __syncthreads();
+      for (int i = t; i < ns * ns * NB * NB; i += nt) {
+        const int b = i % NB, a = (i / NB) % NB, blk = i / (NB * NB), sa = blk >> 1, sb = blk & 1;
+        const int na = nodes[f.face[sa] * NB + a], nb = nodes[f.face[sb] * NB + b];
+        const bool on_a = na >> 4 == side_bit[sa] * P, on_b = nb >> 4 == side_bit[sb] * P;
+        const int ca = na & 15, cb = nb & 15;
+        const double v = on_a && on_b ? XB[(blk * NBF + ca) * NBF + cb]
+                         : on_a       ? X[(blk * NBF + ca) * NB + (nb >> 4) * NBF + cb]
+                         : on_b       ? fp.tau * X[(((sb << 1) | sa) * NBF + cb) * NB + (na >> 4) * NBF + ca]
+                                      : 0.0;
+        double* out = sa != sb ? fp.values + pt->out.base[sa] + int64_t(a) * pt->out.len[sa]
+                      : f.interior ? static_cast<double*>(fp.fblk) + (f.i * 2 + sa) * NB * NB + a * NB
+                                   : static_cast<double*>(fp.bblk) + f.i * NB * NB + a * NB;
+        out[b] = v;
+      }
+    }
+    __syncthreads();
+  }
+}
+
 // The facet kernel of the FP64 form: as k_dg_facets, with the products in
 // fixed point (fe_fixed.cuh) and only over face nodes. The normal derivative of
 // a shape function b = (layer m along the face's normal axis, face node c') at
@@ -764,7 +882,8 @@ __device__ __forceinline__ void facet_points_fixed(const FacetParams& fp, int64_
 //   A = sum_q phi_c dS cn phi_c',  B = sum_q phi_c dS (cs d_s + ct d_t) phi_c',
 // and the values of phi and its tangential derivatives are those of one face
 // rule, the points of the other side permuted (a face symmetry). Steps of the
-// product warps:
+// product warps (a facet whose weights leave 2^-872 .. 2^878, or are not finite, is
+// left to odd_facets):
 //   1. right-hand operands (side, point, face node): dS cn phi, dS (cs d_s phi +
 //      ct d_t phi), dS phi as 59-bit integers;
 //   2. per (block, c, c') the three sums over the points, each converted to a
@@ -776,12 +895,13 @@ __device__ __forceinline__ void facet_points_fixed(const FacetParams& fp, int64_
 // bound by the FP64 pipe (67 %: the point data, about 90 operations per facet,
 // and step 2's products with D_m) and issue (60 %).
 template <int P>
-__global__ void __launch_bounds__(128) k_dg_facets_fixed(FacetParams fp) {
+__global__ void __launch_bounds__(128, P == 1 ? 8 : P == 2 ? 7 : 3) k_dg_facets_fixed(const __grid_constant__ FacetParams fp) {
   using L = FixedFacetLayout<P>;
   constexpr int N1 = L::N1, NB = L::NB, NQF = L::NQF, NBF = L::NBF, NT = 96;
   constexpr int NW = 3, NBJ = (NB + 31) / 32;
   extern __shared__ __align__(16) unsigned char sm[];
   __shared__ double aco[42];
+  __shared__ int any_odd;
   using Points = typename L::Points;
   constexpr size_t PTB = (sizeof(Points) + 15) & ~size_t(15);
   int2* tab = reinterpret_cast<int2*>(sm + L::TAB);  // 59-bit phi; 60-bit phi, d_s phi, d_t phi
@@ -796,6 +916,7 @@ __global__ void __launch_bounds__(128) k_dg_facets_fixed(FacetParams fp) {
   const double tau = fp.tau;
   const bool symmetric = __double_as_longlong(tau) == 0x3ff0000000000000ll;  // tau == 1
   for (int i = threadIdx.x; i < 4 * NQF * NBF; i += 128) tab[i] = fp.fix[i];
+  if (threadIdx.x == 0) any_odd = 0;
   for (int i = threadIdx.x; i < 2 * N1; i += 128) Dn[i] = fp.fix_dn[i];
   for (int i = threadIdx.x; i < 6 * NB; i += 128) nodes[i] = face_node<N1>(i / NB, i % NB);
   if (warp == 3 && blockIdx.x < n_fac)
@@ -809,7 +930,9 @@ __global__ void __launch_bounds__(128) k_dg_facets_fixed(FacetParams fp) {
     } else {
       const Points* pt = reinterpret_cast<const Points*>(sm + L::PT + buf * PTB);
       const FacetRef f = facet_ref(fp, id);
-      const int ns = f.ns;
+      const bool odd = pt->odd;
+      if (odd && t == 0) any_odd = 1;
+      const int ns = odd ? 0 : f.ns;  // (0: nothing to do here, the facet is left to odd_facets)
       // 1. right-hand operands
       for (int i = t; i < ns * NQF * NBF; i += NT) {
         const int c = i % NBF, sq = i / NBF, side = sq / NQF, q = sq % NQF;
@@ -829,7 +952,6 @@ __global__ void __launch_bounds__(128) k_dg_facets_fixed(FacetParams fp) {
       }
       product_barrier();
       // 2. the sums over the points
-      const bool odd = pt->odd;
       for (int i = t; i < ns * ns * NBF * NBF; i += NT) {
         const int c2 = i % NBF, rest = i / NBF, c = rest % NBF, blk = rest / NBF, sa = blk >> 1, sb = blk & 1;
         FixAcc<30> a, b, y;
@@ -852,10 +974,9 @@ __global__ void __launch_bounds__(128) k_dg_facets_fixed(FacetParams fp) {
         // X scaled by -s_a / 2 (boundary: -1), Y by s_a s_b
         const int h = f.interior ? 1 : 0;
         const int64_t ia = a.get(ga), ib = b.get(gb), iy = y.get(gy);
-        double A = fix_to_double(sa ? ia : -ia, fix_exponent(pt->ew[sb][0] + 2 * fp.fix_lp - 56 - ga - h));
-        double Bt = fix_to_double(sa ? ib : -ib, fix_exponent(pt->ew[sb][1] + fp.fix_lp + fp.fix_ld - 56 - gb - h));
-        double Yv = fix_to_double(sa == sb ? iy : -iy, fix_exponent(pt->ey + 2 * fp.fix_lp - 56 - gy));
-        if (odd) A = Bt = Yv = __longlong_as_double(0x7ff8000000000000ll);
+        const double A = fix_to_double(sa ? ia : -ia, fix_exponent(pt->ew[sb][0] + 2 * fp.fix_lp - 56 - ga - h));
+        const double Bt = fix_to_double(sa ? ib : -ib, fix_exponent(pt->ew[sb][1] + fp.fix_lp + fp.fix_ld - 56 - gb - h));
+        const double Yv = fix_to_double(sa == sb ? iy : -iy, fix_exponent(pt->ey + 2 * fp.fix_lp - 56 - gy));
         const int fs = sb ? f.face[1] % 2 : f.face[0] % 2;  // the face layer of side sb
         double* x = X + (blk * NBF + c) * NB + c2;
 #pragma unroll
@@ -904,7 +1025,7 @@ __global__ void __launch_bounds__(128) k_dg_facets_fixed(FacetParams fp) {
             for (int j = 0; j < NBJ; ++j) {
               const double* src = face_row ? on[j] + ca * stride[j] : off[j] + ma * NBF + ca;
               double v = face_row || bon[j] ? *src : 0.0;
-              if (!decltype(unit)::value && !face_row) v *= tau;
+              if (!decltype(unit)::value && !face_row && bon[j]) v *= tau;
               if (NB % 32 == 0 || lane + 32 * j < NB) out[32 * j] = v;
             }
           }
@@ -915,6 +1036,7 @@ __global__ void __launch_bounds__(128) k_dg_facets_fixed(FacetParams fp) {
     }
     __syncthreads();
   }
+  if (any_odd) odd_facets<P>(fp, sm, aco);  // (after the loop: a call among its steps costs them registers)
 }
 
 }  // namespace dg

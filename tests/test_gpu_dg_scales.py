@@ -53,3 +53,44 @@ def test_graded_layers(order, scrambled, ratio):
         torch.cuda.synchronize()
         assert row_scaled_error(rp, col, v.cpu().numpy(), val.astype(np.float64)) <= TOL
     g.close()
+
+
+@pytest.mark.parametrize("order", [1, 2, 3])
+@pytest.mark.parametrize("tau", [1.0, -0.7])
+def test_weights_outside_the_fixed_point_range(order, tau):
+    """Cells of thickness t = 2^-900: the weights through their faces are 2^900, those through their sides 2^-900. Up
+    to parts t^2 of an entry the matrix is 1/t times a fixed one, which t = 2^-300 (in range) gives as well."""
+    vals = {}
+    for k in (300, 900):
+        t = 2.0**-k
+        g = feasm.DGSpace(layers(order, [0.0, t, 2 * t, 3 * t]), order)
+        v, _ = g.assemble(tau, 12.0, 2.0, prec="fp64")
+        rp, col = (x.cpu().numpy() for x in g.pattern())
+        vals[k] = np.ldexp(v.cpu().numpy(), -k)
+        if k == 300:
+            ref = dg_values(layers(order, [0.0, t, 2 * t, 3 * t]), order, tau, 12.0, g.facets(), rp, col)
+            ref = np.ldexp(ref, -300).astype(np.float64)
+            assert row_scaled_error(rp, col, vals[k], ref) <= TOL
+        g.close()
+    assert np.isfinite(vals[900]).all() and row_scaled_error(rp, col, vals[900], ref) <= TOL
+
+
+def test_nan_position_reaches_its_facets_only():
+    mesh = layers(2, [0.0, 1.0, 2.0, 3.0])
+    g = feasm.DGSpace(mesh, 2)
+    want, _ = g.assemble(1.0, 12.0, 2.0, prec="fp64")
+    g.close()
+    coords = np.array(mesh.coords)
+    coords[0] = np.nan  # a corner of cell 0
+    g = feasm.DGSpace(inputs.Mesh(coords, mesh.cell_vertices, mesh.shape, mesh.extent), 2)
+    got, _ = g.assemble(1.0, 12.0, 2.0, prec="fp64")
+    rp, col = (x.cpu().numpy() for x in g.pattern())
+    plus, minus, *_ = g.facets()
+    g.close()
+    got, want = got.cpu().numpy(), want.cpu().numpy()
+    rows = np.repeat(np.arange(rp.size - 1), np.diff(rp))
+    near = np.isin(np.arange(mesh.n_cells), np.concatenate([[0], minus[plus == 0], plus[minus == 0]]))
+    far = ~near[rows // 27] & ~near[col // 27]
+    assert far.any() and np.array_equal(got[far], want[far]) and np.isnan(got).any()
+    own = (rows // 27 == 0) & (col // 27 == 0)
+    assert not np.isfinite(got[own]).any()
