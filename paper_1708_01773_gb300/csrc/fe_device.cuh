@@ -397,7 +397,7 @@ __device__ __forceinline__ bool cell_block_fixed(const CellParams& prm, int64_t 
         s.add(C[3 * k + 1], d1);
         s.add(C[3 * k + 2], d2);
         const int sh = min(60 - B + sexp[c * 4 + (NC == 1 ? 0 : k)] - ((pack >> (9 * k)) & 0x1ff), 62);
-        g[i * 3 + k] = fix_limbs<LOLO ? 32 : 30>(((s.get() >> (sh - 1)) + 1) >> 1);
+        g[i * 3 + k] = fix_limbs<LOLO ? 32 : 30>(s.get_shifted(sh));
       }
     }
   };

@@ -946,9 +946,9 @@ __global__ void __launch_bounds__(128, P == 1 ? 8 : P == 2 ? 7 : 3) k_dg_facets_
         b.add(pt->w[side][q][1], ps);
         b.add(pt->w[side][q][2], pq);
         y.add(pt->ds[q], ph);
-        R[i * 3] = fix_limbs<30>((a.get() + 1) >> 1);
-        R[i * 3 + 1] = fix_limbs<30>((b.get() + 1) >> 1);
-        R[i * 3 + 2] = fix_limbs<30>((y.get() + 1) >> 1);
+        R[i * 3] = fix_limbs<30>(a.get_shifted(1));
+        R[i * 3 + 1] = fix_limbs<30>(b.get_shifted(1));
+        R[i * 3 + 2] = fix_limbs<30>(y.get_shifted(1));
       }
       product_barrier();
       // 2. the sums over the points

@@ -72,8 +72,11 @@ struct FixAcc {
     hh += x >> L;
     x &= (int64_t(1) << L) - 1;
   }
-  // value / 2^(2L), rounded
-  __device__ __forceinline__ int64_t get() const { return hh + ((x + (int64_t(1) << (L - 1))) >> L); }
+  // value / 2^(2L + sh), 1 <= sh <= 62, rounded to nearest from the sum's full
+  // length. (Rounded to 2L first, half of all values are ties where one more bit
+  // goes; rounding those up moves every operand the same way, by a quarter unit on
+  // average, and leaves a residual of translations in every cell.)
+  __device__ __forceinline__ int64_t get_shifted(int sh) const { return (((hh + (x >> L)) >> (sh - 1)) + 1) >> 1; }
   // After drain(): adds an exact sum of lo lo products
   __device__ __forceinline__ void add_low(int64_t lolo) {
     x += (lolo + (int64_t(1) << (L - 1))) >> L;
