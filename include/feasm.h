@@ -332,6 +332,14 @@ void fe_batch_destroy(fe_batch* b);
  * Asynchronous on `stream`; FE_ERR_INVALID_ARG for NULL buffers with n > 0. */
 int fe_selftest_conversions(const double* x, int64_t n, float* out32, double* out64, void* stream);
 
+/* Self-test of the FP64 arithmetic that the library does on the FP32 and integer
+ * pipes. For device inputs x[i] and v[i], i < n, with y = x[(i + 1) % n], writes
+ * out[5 i + 0..4] = 1 / x; 1 / sqrt(x) for positive normal x (NaN for others);
+ * x and x + y through the scatter's integer accumulator (by the hardware where
+ * that leaves them to the general sum); v 2^-60, ties away from zero.
+ * Asynchronous on `stream`; FE_ERR_INVALID_ARG for NULL buffers with n > 0. */
+int fe_selftest_arithmetic(const double* x, const int64_t* v, int64_t n, double* out, void* stream);
+
 /* ------------------------------------------------------------------------
  * Strong Dirichlet conditions (paper, Sect. "Strong imposition of boundary
  * conditions", Eq. dirichlet_bc_discrete_problem). The DOFs of a space split

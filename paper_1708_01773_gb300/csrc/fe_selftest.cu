@@ -50,8 +50,36 @@ __global__ void k_selftest_conversions(const double* x, int64_t n, float* out32,
   }
 }
 
+// The FP64 arithmetic that runs on the FP32 and integer pipes instead: for each x
+// and its successor y in the array, and the integer v.
+__global__ void k_selftest_arithmetic(const double* x, const int64_t* v, int64_t n, double* out) {
+  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double a = x[i], b = x[i + 1 < n ? i + 1 : 0];
+  double* o = out + i * 5;
+  o[0] = reciprocal(a);
+  int k2 = 0;
+  bool odd = false;
+  const double y = fix_rsqrt(a, k2, odd);
+  o[1] = odd ? __longlong_as_double(0x7ff8000000000000ll) : fix_scale2(y, -k2);
+  FxChain c = FxChain::term(a);
+  o[2] = c.odd() ? a : c.round();
+  c.add(FxChain::term(b));
+  o[3] = c.odd() ? __dadd_rn(a, b) : c.round();
+  o[4] = fix_to_double(v[i], fix_exponent(-60));
+}
+
 }  // namespace
 }  // namespace feasm
+
+extern "C" int fe_selftest_arithmetic(const double* x, const int64_t* v, int64_t n, double* out, void* stream) {
+  if (n < 0 || (n > 0 && (!x || !v || !out))) return feasm::set_error(FE_ERR_INVALID_ARG, "invalid self-test buffers");
+  if (n == 0) return FE_OK;
+  const int64_t blocks = (n + 255) / 256;
+  feasm::k_selftest_arithmetic<<<unsigned(blocks), 256, 0, static_cast<cudaStream_t>(stream)>>>(x, v, n, out);
+  const cudaError_t e = cudaGetLastError();
+  return e == cudaSuccess ? FE_OK : feasm::set_error(FE_ERR_CUDA, cudaGetErrorString(e));
+}
 
 extern "C" int fe_selftest_conversions(const double* x, int64_t n, float* out32, double* out64, void* stream) {
   if (n < 0 || (n > 0 && (!x || !out32 || !out64)))

@@ -67,3 +67,26 @@ def test_overlapped_scatter_in_a_row_and_captured(order, problem, shape, prec):
         assert torch.equal(got_v, want_v) and torch.equal(got_r, want_r)
     assert sp.status() == 0
     sp.close()
+
+
+def shapes_around(rows):
+    """The Q1 elasticity bricks of nearly equal sides with the most rows up to `rows` and the fewest above."""
+    sizes = sorted((3 * (a + 1) * (b + 1) * (c + 1), (a, b, c)) for a in range(16, 40) for b in range(a, a + 3)
+                   for c in range(b, b + 3))
+    return [s for s in sizes if s[0] <= rows][-1][1], [s for s in sizes if s[0] > rows][0][1]
+
+
+@pytest.mark.parametrize("above", [False, True])
+def test_node_rows_on_both_sides_of_the_rule(above):
+    """Q1 elasticity, whose larger systems take the three rows of a node together, at 320 rows per SM."""
+    shape = shapes_around(320 * torch.cuda.get_device_properties(0).multi_processor_count)[above]
+    prob = inputs.small_problem(shape, 1, 1, seed=302)
+    rp, col, val, rhs = oracle.assemble_csr(prob)
+    sp = feasm.FESpace(prob)
+    coef = torch.tensor(prob.coef, device="cuda")
+    for prec in ("fp32", "fp64", "bf16"):
+        v, r = sp.assemble(coef, prec=prec)
+        torch.cuda.synchronize()
+        assert row_scaled_error(rp, col, v.cpu().numpy(), val) <= TOL[prec]
+        assert vec_error(r.cpu().numpy(), rhs) <= 1e-12
+    sp.close()
