@@ -65,9 +65,11 @@ typedef enum { FE_POISSON = 0, FE_ELASTICITY = 1, FE_STOKES = 2 } fe_problem;
 /* Arithmetic of the cell-matrix contraction. The geometry (Jacobian,
  * determinant, cofactors) and the global CSR accumulation are always FP64.
  *   FE_PREC_FP64: FP64 operands; the products and sums of a cell matrix in
- *     59-bit fixed point with exact integer sums (errors at or below those of
- *     FP64 products; cells whose numbers fit no common scale are integrated in
- *     plain FP64).
+ *     59-bit fixed point with exact integer sums (cells whose numbers fit no
+ *     common scale are integrated in plain FP64). Measured against extended
+ *     precision, whole matrices in the 2-norm: 5.7e-16 to 9.2e-16 on distorted
+ *     meshes of Q1 to Q3, where FP64 products give 6.1e-16 to 9.6e-16; on
+ *     uniform Q1 elasticity bricks 8.0e-16 to 8.1e-16 after 7.8e-16 to 7.9e-16.
  *   FE_PREC_FP32: FP32 operands and FP32 accumulation of the contraction.
  *   FE_PREC_BF16: BF16 operands, FP32 accumulation. */
 typedef enum { FE_PREC_FP64 = 0, FE_PREC_FP32 = 1, FE_PREC_BF16 = 2 } fe_precision;

@@ -234,12 +234,15 @@ __device__ __noinline__ void cell_block_plain(const CellParams& prm, int64_t e0,
 //      coefficient and the elasticity law in integers, one conversion to
 //      double per entry, stored to (a, b) and (b, a). The lo lo products are
 //      in the sums that hold squares for a = b: left out there they lower the
-//      diagonal by 2^-57 of itself in every cell, which a clamped beam of
-//      31 x 21 x 19 cells shows as 1e-12 in its displacement (2e-14 with
-//      them);
+//      diagonal by 6e-17 of itself in every cell (displacement of a clamped
+//      uniform beam of 16 x 9 x 8 cells, against extended precision: 1.0e-14
+//      with them, 1.2e-13 without, 5.0e-14 with FP64 products; of 31 x 21 x 19
+//      cells 1.9e-13, 1.7e-13 and 3.1e-13: few distinct entries, so that their
+//      roundings do not average out);
 //   4. cell vectors in FP64.
 // Bound by: the integer multiply-adds of step 3 (IMAD.WIDE, 25 to 32 lanes per
-// clock per SM) and the conversions to double; FP64 pipe a quarter busy.
+// clock per SM) and the conversions to double (ALU pipe 54 % busy in Q1
+// elasticity, 47 % in Q2; FP64 pipe 35 % and 8 %).
 // Measured against the FP64 multiply-adds (cell_block_plain), ms: Poisson Q1
 // 64^3 2.01 -> 0.42, Q2 32^3 7.44 -> 0.86, Q3 24^3 39.1 -> 4.4; elasticity Q1
 // 64^3 4.31 -> 0.74, Q2 24^3 6.47 -> 0.77, Q3 12^3 10.2 -> 1.13. Error in the

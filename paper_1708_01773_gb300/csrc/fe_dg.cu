@@ -721,8 +721,8 @@ __device__ __forceinline__ void facet_weights_fp64(const FacetParams& fp, const 
 
 // Point data of facet id for the fixed-point products (all 32 lanes of the
 // point warp): the geometry of facet_points, the weights dS cof^T n / det as
-// integers under one scale per side and kind of axis, dS under one, and each point's index in the sides' own
-// face rules.
+// integers under one scale per side and kind of axis, dS under one, and each
+// point's index in the sides' own face rules.
 template <int P>
 __device__ __forceinline__ void facet_points_fixed(const FacetParams& fp, int64_t id, typename FixedFacetLayout<P>::Points* b,
                                                    double* aco, int lane) {
@@ -891,9 +891,12 @@ static __device__ __noinline__ void odd_facets(const FacetParams& fp, unsigned c
 //   3. the entries between face nodes: X + tau X^T + gamma/|F| Y;
 //   4. the blocks, row (block, a), column b.
 // Against FP64 multiply-adds over all nb columns (18,800 per interior facet at
-// p = 2 on a pipe of 2 lanes per clock per SM) 6.0 -> 1.35 ms on 32^3 Q2 cells;
-// bound by the FP64 pipe (67 %: the point data, about 90 operations per facet,
-// and step 2's products with D_m) and issue (60 %).
+// p = 2 on a pipe of 2 lanes per clock per SM) 6.0 -> 1.37 ms on 32^3 Q2 cells;
+// bound by the FP64 pipe (62 %: the point data, about 90 operations per facet,
+// and step 2's products with D_m) and issue (55 %).
+// Blocks per SM: p = 1 as many as 64 registers let in (assembly of 40^3 cells 1.84
+// ms with 8, 1.94 with 7, 2.30 with 5), p = 2 seven of 72 registers (32^3 cells 2.64
+// ms, 2.69 with 8, 2.68 with 6), p = 3 the three that fit the shared memory.
 template <int P>
 __global__ void __launch_bounds__(128, P == 1 ? 8 : P == 2 ? 7 : 3) k_dg_facets_fixed(const __grid_constant__ FacetParams fp) {
   using L = FixedFacetLayout<P>;

@@ -86,8 +86,8 @@ cudaError_t launch_scatter_pattern(const fe_space* s, const ScatterPattern& pt, 
 struct ScatterParams;
 cudaError_t launch_scatter_slots64(const fe_space* s, ScatterParams p, bool node_rows, int64_t max_row_nnz,
                                    int blocks_needed, cudaStream_t st, bool* taken);
-// Systems with at most one row per resident warp (and at most 32 cells around a
-// DOF): the scatter with one row per warp, in every precision.
+// Systems of at most 320 rows per SM (and at most 32 cells around a DOF): the
+// scatter with one row per warp, in every precision.
 cudaError_t launch_scatter_small(const fe_space* s, ScatterParams p, fe_precision prec, int64_t max_row_nnz,
                                  cudaStream_t st, bool* taken);
 // The scatter of rows [r0, r1) only (r0, r1 multiples of the rows per item of

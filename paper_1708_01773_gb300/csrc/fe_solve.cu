@@ -16,7 +16,7 @@
 // grid of 1216 blocks, launched from the host with a look at the residual every
 // 8 iterations, a small system spent most of its time in launches and in
 // summing 1216 partials per block. Measured per iteration, us: 811,200 rows 230 ->
-// 183 (FP64 pipe and HBM), 136,000 rows 77 -> 49, 41,000 rows 48 -> 24, 3,900 rows
+// 183 (FP64 pipe and HBM), 136,000 rows 77 -> 49, 41,000 rows 48 -> 23.4, 3,900 rows
 // 43 -> 15 (latency of the exchanges and of dependent FP64 operations).
 #include <cuda_runtime.h>
 
@@ -247,9 +247,8 @@ __device__ __forceinline__ double quotient(double a, double b, double inv_b) {
 // check (every kCheckEvery iterations) that finds ||r|| <= rtol ||b|| or a
 // matrix that is not positive definite, and at once where p.q, r.z or r.r is not
 // finite: such a sum does not recover, and no later residual may pass for a
-// converged one. Cooperative
-// launch: every block is resident. Virtual block vb owns rows
-// [n vb / nv, n (vb + 1) / nv).
+// converged one. Cooperative launch: every block is resident. Virtual block vb
+// owns rows [n vb / nv, n (vb + 1) / nv).
 //
 // GB300 issues FP64 at 2 lanes per clock per SM and charges a warp instruction
 // in full (64 clocks of its sub-partition) whatever its active lanes; that
@@ -258,14 +257,16 @@ __device__ __forceinline__ double quotient(double a, double b, double inv_b) {
 //              rows), each lane summing every G-th nonzero, then a log2(G)-step
 //              xor butterfly. G = 4 takes the 81 entries of an interior Q1
 //              elasticity row in 21 rounds with 3 idle slots; G = 2 where that
-//              lets a block's 257 to 512 rows run in one pass of its 32 warps;
-//              8 for rows of more than 128 entries;
+//              lets a block's 257 to 512 rows run in one pass of its 32 warps
+//              (Q1 elasticity, us per iteration with G = 2 / 4: 270 rows a block
+//              23.4 / 24.8, 376 rows 26.7 / 26.7, 494 rows 29.2 / 28.9; Poisson,
+//              323 rows 19.0 / 19.5); 8 for rows of more than 128 entries;
 //   sums       the threads' values go through shared memory to one warp per sum
 //              (butterflies in all 32 warps: 160 warp additions a sum);
 //   scalars    alpha and beta in one thread.
 // RES: at most one row per thread (n <= 152 x 1024): x, r, p and D^-1 of the row
 // stay in the thread's registers from iteration to iteration, q in shared
-// memory; only p goes to memory. 41,000 rows: 27 -> 24 us per iteration, of which the SpMV
+// memory; only p goes to memory. 41,000 rows: 27 -> 23.4 us per iteration, of which the SpMV
 // takes 13k of 49k clocks (11k at the FP64 pipe's rate) and the three exchanges
 // 7k to 9k each (a store, its way through L2 to 152 pollers, nine dependent FP64
 // additions).
