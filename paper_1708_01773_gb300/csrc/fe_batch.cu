@@ -121,6 +121,7 @@ __device__ void row_exact64(const ScatterParams& p, int64_t r, int lane, int64_t
   if (p.rhs != nullptr && lane == 0)
     p.rhs[r] = fx_sum<double>(ns, [&](int t) { return __ldcg(p.fe + p.slots[s0 + t]); });
   const int64_t k0 = p.row_ptr[r], k1 = p.row_ptr[r + 1];
+  const int flip = FxChain::flip_of(ns > 0 ? p.slots[s0] : 0);
   int64_t c = p.code_ptr[r];
   for (int64_t kb = k0; kb < k1; kb += 32) {
     const int64_t k = kb + lane;
@@ -138,9 +139,9 @@ __device__ void row_exact64(const ScatterParams& p, int64_t r, int lane, int64_t
         const unsigned code = cp[t];
         return __ldcg(ke + sbase[(code >> 8) & 127u] + (code & 255u));
       };
-      FxChain v = FxChain::term(get(0));  // as k_scatter_slots64, bit for bit
-      for (int t = 1; t < n; ++t) v.add(FxChain::term(get(t)));
-      p.values[k] = v.odd() ? fx_sum<double>(n, get) : v.round();
+      FxChain v = FxChain::term(get(0), flip);  // as k_scatter_slots64, bit for bit
+      for (int t = 1; t < n; ++t) v.add(FxChain::term(get(t), flip));
+      p.values[k] = v.odd() ? fx_sum<double>(n, get) : v.round(flip);
     }
     c += total;
   }

@@ -750,28 +750,41 @@ __device__ __forceinline__ double fx_sum_regs(const double (&v)[N]) {
 // integer S with an exponent e (value S 2^(e - 1080)); a term is its mantissa
 // shifted left by 5 (leading bit at bit 57, room for 32 terms), and the smaller
 // of accumulator and term is shifted right to the larger exponent before the
-// integer addition. Bits lost are below 2^-57 of the largest term so far.
+// integer addition. Bits lost are below 2^-57 of the largest term so far. The
+// shift rounds down, which would be a bias if every sum of a matrix did so (with
+// coefficients that differ by 2^8 and more between cells the sum of all entries
+// was up to 3.8 times what independent roundings allow; cut off towards zero
+// still 1.8 times, as the diagonal has more terms than the others). So half of
+// the rows, by a hash of the first cell-matrix row they sum (the same in every
+// pattern that keeps the row), sum the negated terms: one instruction per term,
+// where rounding each shift would take four.
 struct FxChain {
   int64_t S;
   int e;
-  __device__ __forceinline__ static FxChain term(double x) {
+  // 0, or -1 where the row whose first slot (cell-matrix row) is `slot` sums the negated terms
+  __device__ __forceinline__ static int flip_of(int slot) { return int(uint32_t(slot) * 0x9e3779b1u) >> 31; }
+  __device__ __forceinline__ static FxChain term(double x, int flip) {
     const int hi = __double2hiint(x), lo = __double2loint(x), eb = (hi >> 20) & 0x7ff;
     const uint32_t mh = uint32_t(hi & 0xfffff) | (eb != 0 ? 0x100000u : 0u);
     const int64_t m = int64_t((uint64_t(__funnelshift_l(uint32_t(lo), mh, 5)) << 32) | (uint32_t(lo) << 5));
-    const int64_t sg = int64_t(hi >> 31);
-    return FxChain{(m ^ sg) - sg, max(eb, 1)};
+    const int64_t sg = int64_t((hi >> 31) ^ flip);
+    return FxChain{(m ^ sg) - sg, eb};  // (denormals: half of their value, but odd() unless nothing of them is left)
   }
   __device__ __forceinline__ void add(const FxChain& t) {
-    const int d = t.e - e;
-    const bool up = d > 0;  // the term has the larger exponent
-    const int64_t big = up ? t.S : S, small = up ? S : t.S;
-    S = big + (small >> min(up ? d : -d, 63));
-    e = up ? t.e : e;
+    const int m = max(e, t.e);
+    S = shift_down(S, m - e) + shift_down(t.S, m - t.e);
+    e = m;
+  }
+  // x / 2^d rounded down, d of any size (shr clamps it, >> in C++ does not)
+  __device__ __forceinline__ static int64_t shift_down(int64_t x, int d) {
+    int64_t r;
+    asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(x), "r"(d));
+    return r;
   }
   // near the ends of the exponent range (infinities, NaN, denormals): the sum is redone with fx_sum
   __device__ __forceinline__ bool odd() const { return (e < 80 && S != 0) || e > 2000; }
-  // rounded to the nearest double (ties to even); not if odd()
-  __device__ __forceinline__ double round() const {
+  // the row's sum rounded to the nearest double (ties to even); not if odd()
+  __device__ __forceinline__ double round(int flip) const {
     const uint64_t s = uint64_t(S >> 63);
     const uint64_t mag = (uint64_t(S) ^ s) - s;
     const int lz = __clzll(static_cast<long long>(mag));
@@ -780,7 +793,7 @@ struct FxChain {
     const uint32_t rem = nl & 0x7ffu, last = (nl >> 11) & 1u;
     uint64_t bits = (uint64_t(uint32_t(63 - lz + e - 1080 + 1022) << 20) << 32) +
                     ((uint64_t(nh >> 11) << 32) | __funnelshift_r(nl, nh, 11)) + (rem + last > 0x400u ? 1u : 0u);
-    bits |= s & 0x8000000000000000ull;
+    bits |= (s ^ uint64_t(int64_t(flip))) & 0x8000000000000000ull;
     return __longlong_as_double(static_cast<long long>(mag == 0 ? 0ull : bits));
   }
 };

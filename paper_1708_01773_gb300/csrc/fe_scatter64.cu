@@ -25,7 +25,7 @@ struct SlotScatter64 {
   template <int B, bool IDX32>
   __device__ __forceinline__ static void batch(const ScatterParams& p, const double* ke, const uint16_t* pos,
                                                int my_slot, int s_begin, int64_t* acc, int* exps, int rs, int dummy,
-                                               int lane) {
+                                               int lane, const int (&flip)[R]) {
     double x[B][CH][R];
     int kk[B][CH];
 #pragma unroll
@@ -53,7 +53,7 @@ struct SlotScatter64 {
         for (int i = 0; i < R; ++i) {
           int64_t* ai = acc + i * rs;
           int* ei = exps + i * rs;
-          FxChain v = FxChain::term(x[t][c][i]);
+          FxChain v = FxChain::term(x[t][c][i], flip[i]);
           if (!first) {
             FxChain acc{ai[k], ei[k]};
             acc.add(v);
@@ -170,17 +170,20 @@ __global__ void __launch_bounds__(kScatterWarps * 32, 4) k_scatter_slots64(Scatt
       c0n = p.code_ptr[rn];
     }
     const uint16_t* pos = p.pos + c0 + lane;
+    int flip[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) flip[i] = FxChain::flip_of(__shfl_sync(kFull, my_slot, 0) + i * S::NBR);
     int sb = 0;
     while (sb < ns) {
       const int left = ns - sb;
       if (S::SB >= 4 && left >= 4) {
-        S::template batch<4, IDX32>(p, ke, pos, my_slot, sb, acc, exps, rs, dummy, lane);
+        S::template batch<4, IDX32>(p, ke, pos, my_slot, sb, acc, exps, rs, dummy, lane, flip);
         sb += 4;
       } else if (S::SB >= 2 && left >= 2) {
-        S::template batch<2, IDX32>(p, ke, pos, my_slot, sb, acc, exps, rs, dummy, lane);
+        S::template batch<2, IDX32>(p, ke, pos, my_slot, sb, acc, exps, rs, dummy, lane, flip);
         sb += 2;
       } else {
-        S::template batch<1, IDX32>(p, ke, pos, my_slot, sb, acc, exps, rs, dummy, lane);
+        S::template batch<1, IDX32>(p, ke, pos, my_slot, sb, acc, exps, rs, dummy, lane, flip);
         sb += 1;
       }
     }
@@ -194,7 +197,7 @@ __global__ void __launch_bounds__(kScatterWarps * 32, 4) k_scatter_slots64(Scatt
       for (int j = lane; j < nnz; j += 32) {
         const FxChain v{acc[i * rs + j], exps[i * rs + j]};
         odd |= v.odd();
-        p.values[ki + j] = v.round();
+        p.values[ki + j] = v.round(flip[i]);
       }
       if (__any_sync(kFull, odd)) {
         __syncwarp();
@@ -253,6 +256,7 @@ __global__ void __launch_bounds__(kScatterWarps * 32) k_scatter_small(ScatterPar
   const int ns = int(p.slot_ptr[r + 1] - s0), nnz = int(p.row_ptr[r + 1] - k0);
   const int my_slot = lane < ns ? p.slots[s0 + lane] : 0;
   const uint16_t* pos = p.pos + c0 + lane;
+  const int flip[1] = {F64 ? FxChain::flip_of(__shfl_sync(kFull, my_slot, 0)) : 0};
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const TK* ke = reinterpret_cast<const TK*>(p.ke) + lane;
   double fe = 0.0;
@@ -263,7 +267,7 @@ __global__ void __launch_bounds__(kScatterWarps * 32) k_scatter_small(ScatterPar
     auto run = [&](auto n) {
       constexpr int B = decltype(n)::value;
       if constexpr (F64)
-        S::template batch<B, true>(p, ke, pos, my_slot, sb, acc64, exps, rs, dummy, lane);
+        S::template batch<B, true>(p, ke, pos, my_slot, sb, acc64, exps, rs, dummy, lane, flip);
       else
         S::template batch<B, true>(p, ke, pos, my_slot, sb, acc, rs, dummy, lane);
       sb += B;
@@ -280,7 +284,7 @@ __global__ void __launch_bounds__(kScatterWarps * 32) k_scatter_small(ScatterPar
     for (int j = lane; j < nnz; j += 32) {
       const FxChain v{acc64[j], exps[j]};
       odd |= v.odd();
-      p.values[k0 + j] = v.round();
+      p.values[k0 + j] = v.round(flip[0]);
     }
     if (__any_sync(kFull, odd)) {
       __syncwarp();

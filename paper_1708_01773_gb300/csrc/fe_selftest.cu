@@ -62,10 +62,11 @@ __global__ void k_selftest_arithmetic(const double* x, const int64_t* v, int64_t
   bool odd = false;
   const double y = fix_rsqrt(a, k2, odd);
   o[1] = odd ? __longlong_as_double(0x7ff8000000000000ll) : fix_scale2(y, -k2);
-  FxChain c = FxChain::term(a);
-  o[2] = c.odd() ? a : c.round();
-  c.add(FxChain::term(b));
-  o[3] = c.odd() ? __dadd_rn(a, b) : c.round();
+  const int flip = FxChain::flip_of(i);
+  FxChain c = FxChain::term(a, flip);
+  o[2] = c.odd() ? a : c.round(flip);
+  c.add(FxChain::term(b, flip));
+  o[3] = c.odd() ? __dadd_rn(a, b) : c.round(flip);
   o[4] = fix_to_double(v[i], fix_exponent(-60));
 }
 

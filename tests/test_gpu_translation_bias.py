@@ -53,3 +53,26 @@ def test_translations_on_the_faces(order, problem, n):
             print(order, problem, axis, side, total, bound, total / bound)
             assert abs(total) <= bound
     sp.close()
+
+
+@pytest.mark.parametrize("order, problem, n", [(1, 0, 64), (1, 1, 48), (2, 0, 24), (2, 1, 16)])
+@pytest.mark.parametrize("contrast", ["2^-8 or 1", "2^-40 or 1", "2^-16 to 1"])
+def test_sum_of_all_entries_with_coefficient_contrast(order, problem, n, contrast):
+    """The scatter's sums lose bits only where their terms differ by more than 2^5, as they do between cells of very
+    different coefficients. All entries together cancel; the bound is the one above. What is cut off (0.4 units of 2^-57
+    of an entry and addition on average) must cancel with them: cut off downwards it is 3.8 times the bound."""
+    prob = inputs.small_problem((n, n, n), order, problem, seed=92)
+    rng = np.random.default_rng(1)
+    cells = prob.coef.size
+    coef = {"2^-8 or 1": np.where(rng.random(cells) < 0.5, 1.0, 2.0**-8),
+            "2^-40 or 1": np.where(rng.random(cells) < 0.5, 1.0, 2.0**-40),
+            "2^-16 to 1": 2.0 ** rng.uniform(-16, 0, cells)}[contrast]
+    sp = feasm.FESpace(prob)
+    v, _ = sp.assemble(torch.tensor(coef, device="cuda"), prec="fp64")
+    k = 61 - int(np.ceil(np.log2(float(v.abs().max()))))
+    scaled = torch.round(torch.ldexp(v, torch.tensor(float(k), dtype=torch.float64, device="cuda"))).to(torch.int64)
+    total = float(scaled.sum()) * 2.0 ** -k
+    bound = 7.5 * 2.0**-53 / 3**0.5 * float(v.norm()) + 2.0**-61 * float(v.abs().sum())
+    print(order, problem, contrast, total, bound, total / bound)
+    assert abs(total) <= bound
+    sp.close()
