@@ -100,10 +100,11 @@ static __device__ __noinline__ void row_from_codes(const ScatterParams& p, int64
 // nonzero. Sums near the ends of the exponent range (infinities, NaN,
 // denormals) are redone with fx_sum over the row's destination-sorted codes.
 // k_scatter_rows gives each nonzero a lane, with two passes over its 1 to 8
-// terms, so that a warp's lanes wait for the one with the most. Bound by the ALU pipe (70 % busy, about 20 integer
-// instructions per term); measured against k_scatter_rows, ms: elasticity Q1
-// 64^3 1.60 -> 0.56, Q2 24^3 0.945 -> 0.378, Q3 12^3 1.20 -> 0.33; Poisson Q1
-// 64^3 0.28 -> 0.195, Q3 24^3 0.54 -> 0.25; Stokes 24^3 1.15 -> 0.42.
+// terms, so that a warp's lanes wait for the one with the most. Bound by the ALU
+// pipe (67 % busy, about 20 integer instructions per term); measured against
+// k_scatter_rows, ms: elasticity Q1 64^3 1.60 -> 0.550, Q2 24^3 0.945 -> 0.367, Q3
+// 12^3 1.20 -> 0.322; Poisson Q1 64^3 0.28 -> 0.182, Q3 24^3 0.54 -> 0.246; Stokes
+// 24^3 1.15 -> 0.41.
 template <int NL, int R, bool IDX32>
 __global__ void __launch_bounds__(kScatterWarps * 32, 4) k_scatter_slots64(ScatterParams p) {
   using S = SlotScatter64<NL, R>;
