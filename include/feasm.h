@@ -479,8 +479,9 @@ void fe_dirichlet_destroy(fe_dirichlet* d);
  * Interior facets take K+ = the lower cell id; each contributes the four
  * blocks (K+K+, K+K-, K-K+, K-K-), row = test function, column = trial
  * function. Facet integrals use (p+1)^2 Gauss points and FP64 geometry; their
- * products are in 59-bit fixed point with exact sums in the FP64 form and in
- * FP32 in the FP32 and BF16 forms.
+ * products are in 59-bit fixed point with exact sums in the FP64 form (in plain
+ * FP64 for facets whose weights leave 2^-872 .. 2^878) and in FP32 in the FP32
+ * and BF16 forms.
  * ------------------------------------------------------------------------ */
 typedef struct fe_dg fe_dg; /* opaque, library-owned */
 

@@ -1,6 +1,6 @@
 // CUDA kernels of libfeasm (sm_103a): cell integration (geometry, physical
-// gradients, cell-matrix contraction, cell vectors), the deterministic
-// segmented scatter into CSR, and the compliance adjoint.
+// gradients, cell-matrix contraction, cell vectors) and the deterministic
+// segmented scatter into CSR.
 #include "fe_device.cuh"
 
 namespace feasm {
